@@ -1054,6 +1054,20 @@ constexpr int kRowCols = 32;
 constexpr int kRowMax = 16;  // rows of a sequence in a commit (n_layers at most)
 constexpr uint32_t kRowSmem = 2 * 2 * 2 * kTcHalfBytes + 2 * kRowCols * 256;
 
+// Sequence b's rows in a block (its rows of the commit are o0 .. o1 - 1): n of them, of which
+// nv, from row lo of the commit at position P on, have a place in the cache.
+struct BlockRows {
+    int n, lo, nv, P;
+};
+
+__device__ __forceinline__ BlockRows block_rows_of(const AttnArgs& a, int o0, int o1, int b, int row0, int block_rows) {
+    const int r0 = max(o0, row0), r1 = min(o1, row0 + block_rows);
+    if (r1 <= r0) return {0, r0, 0, 0};
+    const int2 in = rows_in_cache(a.prefix_len[b], o1 - o0, a.max_seq);
+    const int lo = max(r0, o0 + in.x), nv = max(min(r1, o0 + in.y) - lo, 0);
+    return {r1 - r0, lo, nv, nv ? a.prefix_len[b] + (lo - o0) : 0};
+}
+
 template <int G>
 __global__ void __launch_bounds__(kAttnWarps * 32, 2) attn_rows_kernel(const AttnArgs a, const int* off, int row0,
                                                                        int block_rows) {
@@ -1069,14 +1083,13 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 2) attn_rows_kernel(const Att
 
     const int s = blockIdx.x % a.n_split, cb = blockIdx.x / a.n_split, g = blockIdx.y, b = blockIdx.z;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    const int o0 = off[b], lo = max(o0, row0), n = min(off[b + 1], row0 + block_rows) - lo;
-    if (n <= 0) {  // no rows of this sequence in the block
+    const BlockRows br = block_rows_of(a, off[b], off[b + 1], b, row0, block_rows);
+    if (br.n <= 0) {  // no rows of this sequence in the block
         griddep_launch_dependents();
         return;
     }
-    const int P = a.prefix_len[b] + lo - o0;  // position of the first row; cached keys before it
-    const int nv = P < 0 ? 0 : min(n, a.max_seq - P);
-    if (nv < n && blockIdx.x == 0 && g == 0 && t == 0) atomicOr(a.status, ST_CAPACITY);
+    const int lo = br.lo, nv = br.nv, P = br.P;  // P: position of the first row; cached keys before it
+    if (nv < br.n && blockIdx.x == 0 && g == 0 && t == 0) atomicOr(a.status, ST_CAPACITY);
     const int t0 = s * a.split, ncol = min(kRowCols, nv * G - cb * kRowCols);
     if (nv <= 0 || ncol <= 0 || t0 > P) {
         griddep_launch_dependents();
@@ -1451,11 +1464,10 @@ __global__ void __launch_bounds__(kAttnWarps * 32) append_rows_kernel(const Attn
     constexpr int HD = 128, HALF = 64;
     const int g = blockIdx.x, b = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     griddep_launch_dependents();
-    const int o0 = off[b], lo = max(o0, row0), n = min(off[b + 1], row0 + block_rows) - lo;
-    const int P = a.prefix_len[b] + lo - o0;
-    const int nv = P < 0 ? 0 : min(n, a.max_seq - P);
+    const BlockRows br = block_rows_of(a, off[b], off[b + 1], b, row0, block_rows);
+    const int lo = br.lo, nv = br.nv, P = br.P;
     griddep_wait();
-    if (nv < n && g == 0 && threadIdx.x == 0) atomicOr(a.status, ST_CAPACITY);
+    if (nv < br.n && g == 0 && threadIdx.x == 0) atomicOr(a.status, ST_CAPACITY);
     for (int i = warp; i < nv; i += kAttnWarps) {
         bf16_t* krow = cache_row<bf16_t>((bf16_t*)a.kc, a, b, g, P + i, HD);
         bf16_t* vrow = cache_row<bf16_t>((bf16_t*)a.vc, a, b, g, P + i, HD);

@@ -31,8 +31,10 @@ cudaError_t launch_commit_gather(const void* feat, const int* tok, const int* n_
 }
 
 // The rows of a whole commit for the multi-row path: one CTA; thread b owns sequence b, b +
-// blockDim, ... The first row of sequence b in its block decides the cached keys all of the
-// block's rows of b share (the rows before it are stored by then), so the splits follow it.
+// blockDim, ... The first row of sequence b in its block that has a place in the cache decides the
+// cached keys all of the block's rows of b share (the rows before it are stored by then), so the
+// splits follow it. Rows without a place have no splits; attn_rows_kernel leaves them out by the
+// same rule (rows_in_cache).
 __global__ void __launch_bounds__(256) commit_plan_kernel(const int* tok, const int* n_rows, const int* prefix_len,
                                                           int B, int L, int block_rows, int split, int max_seq,
                                                           int* off, int* total, int* x_row, int* ctok, int* nact) {
@@ -56,12 +58,13 @@ __global__ void __launch_bounds__(256) commit_plan_kernel(const int* tok, const 
         base = so[256];
         if (b < B) {
             const int o = so[t], P = prefix_len[b];
+            const int2 in = rows_in_cache(P, n, max_seq);
             off[b] = o;
             for (int i = 0; i < n; ++i) {
-                const int r = o + i, first = max(o, r / block_rows * block_rows), P0 = P + first - o;
+                const int r = o + i, first = max(o + in.x, r / block_rows * block_rows) - o;
                 x_row[r] = b * L + i;
                 ctok[r] = tok[(size_t)b * L + i];
-                nact[r] = P0 >= 0 && P + i + 1 <= max_seq ? P0 / split + 1 : 0;
+                nact[r] = i >= in.x && i < in.y ? (P + first) / split + 1 : 0;
             }
         }
         __syncthreads();

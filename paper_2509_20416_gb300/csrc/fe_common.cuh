@@ -85,6 +85,16 @@ struct LaunchStamp {
     }
 };
 
+// ---- the rows of a commit --------------------------------------------------------------
+// Of a sequence's rows 0 .. n - 1 at positions prefix + row, those with a place in a cache of
+// max_seq positions: x .. y - 1 (x = y when there are none). In 64 bits: prefix_len is device data
+// and may hold anything.
+__device__ __forceinline__ int2 rows_in_cache(int prefix, int n, int max_seq) {
+    const long long first = min(max(-(long long)prefix, 0ll), (long long)n);
+    const long long end = min(max((long long)max_seq - prefix, first), (long long)n);
+    return make_int2((int)first, (int)end);
+}
+
 // ---- mbarrier -------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return (uint32_t)__cvta_generic_to_shared(p);
