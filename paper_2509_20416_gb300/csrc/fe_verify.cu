@@ -233,12 +233,19 @@ __global__ void __launch_bounds__(kVsThreads) verify_sampled_kernel(const Verify
 // thread and one exchange: every warp sends its partial total to every CTA through
 // distributed shared memory (st.async, completing on the receiver's mbarrier) and sums all of
 // them itself. Every warp takes every decision itself, too, from the same values, with child j
-// of the node on its lane j; there is no other synchronisation in the walk. Sums are float32
-// pairs (2^-48), the same accuracy as compensated float shares added in double, and the two
-// scales 1 / Z and 1 / (1 - drawn mass) are rounded once from pairs. Elementwise arithmetic is
-// verify_sampled_kernel's; a token that was drawn leaves s by zeroing its owner's q.
+// of the node on its lane j; there is no other synchronisation in the walk. Elementwise
+// arithmetic is verify_sampled_kernel's; a token that was drawn leaves s by zeroing its owner's
+// q. The sums (double there):
+//   - Z: compensated float shares of E entries, added as float pairs (2^-48; the shares there,
+//     of V / 512 entries, are the larger error of the two);
+//   - the drawn mass and the CDF of the bonus draw: 64-bit fixed point in units of 2^-62, which
+//     holds a float32 of 2^-39 or more exactly (smaller ones to a unit). Integer sums do not
+//     depend on their order, so the totals of CTAs, segments and entries agree to the last
+//     bit and the draw never falls between two of them.
 // 4 sequences, 128256 entries, 6 levels x 8 candidates: 324 us on one CTA each; here 28 us with
-// the totals added in double by one warp between CTA barriers, 25 without.
+// the totals added in double by one warp between CTA barriers, 25.3 with every total a float
+// pair (whose CDF could pick an entry next to its own, even one of probability 0, when the
+// deviate lay within 2^-48 of a CDF edge), 25.9 in fixed point.
 struct FF {  // an unevaluated sum of two floats
     float h = 0.f, l = 0.f;
 };
@@ -259,23 +266,48 @@ __device__ __forceinline__ FF ff_shfl_xor(FF a, int o) {
     return r;
 }
 
-__device__ __forceinline__ double ff_value(FF a) { return (double)a.h + (double)a.l; }
+// A probability in units of 2^-62, rounded down: its 24 bits shifted to their place. Taken into
+// [0, 2) first (0 for a NaN); sums saturate (one of 2 or more is above every deviate).
+using fx64 = unsigned long long;
+constexpr fx64 kFxOne = 1ull << 62;
+
+__device__ __forceinline__ float fx_clamp(float w) { return fminf(fmaxf(w, 0.f), 1.9999999f); }
+
+__device__ __forceinline__ fx64 fx(float w) {
+    const uint32_t u = __float_as_uint(fx_clamp(w));
+    fx64 r;  // (shr clamps its count: 0 from 64 on)
+    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"((fx64)((u & 0x7fffffu) | 0x800000u) << 39), "r"(127u - (u >> 23)));
+    return r;
+}
+
+__device__ __forceinline__ fx64 fx_add(fx64 a, fx64 b) { return a + b < a ? ~0ull : a + b; }
+
+// 1 / (a 2^-62), a > 0, rounded once from a remainder known to ~2^-49: a is split into three
+// floats, and the remainder of the first one's reciprocal is exact
+__device__ __forceinline__ float fx_rcp(fx64 a) {
+    constexpr float kUnit = 1.f / (float)kFxOne;
+    const float h = __ull2float_rn(a);
+    const long long d = (long long)(a - __float2ull_rn(h));  // (|d| < 2^39)
+    const float l = __ll2float_rn(d), l2 = __ll2float_rn(d - __float2ll_rn(l));
+    const float r = __frcp_rn(h * kUnit);
+    return fmaf(r, fmaf(-r, l2 * kUnit, fmaf(-r, l * kUnit, fmaf(-r, h * kUnit, 1.f))), r);
+}
 
 // Transposing warp reduction: afterwards lane l holds, in v[0], the warp-wide sum of value
 // l >> (5 - log2 E).
 template <int N, int O>
-__device__ __forceinline__ void ff_multi_sum(FF* v, int lane) {
+__device__ __forceinline__ void fx_multi_sum(fx64* v, int lane) {
     if constexpr (N > 1) {
         const bool upper = (lane & O) != 0;
 #pragma unroll
         for (int i = 0; i < N / 2; ++i) {
-            const FF send = upper ? v[i] : v[i + N / 2], keep = upper ? v[i + N / 2] : v[i];
-            v[i] = ff_add(keep, ff_shfl_xor(send, O));
+            const fx64 send = upper ? v[i] : v[i + N / 2], keep = upper ? v[i + N / 2] : v[i];
+            v[i] = fx_add(keep, __shfl_xor_sync(0xffffffffu, send, O));
         }
-        ff_multi_sum<N / 2, O / 2>(v, lane);
+        fx_multi_sum<N / 2, O / 2>(v, lane);
     } else {
 #pragma unroll
-        for (int o = O; o >= 1; o >>= 1) v[0] = ff_add(v[0], ff_shfl_xor(v[0], o));
+        for (int o = O; o >= 1; o >>= 1) v[0] = fx_add(v[0], __shfl_xor_sync(0xffffffffu, v[0], o));
     }
 }
 
@@ -295,12 +327,12 @@ __device__ __forceinline__ void cluster_sync() {
 }
 
 // 16 bytes into CTA `rank`'s copy of `slot`, completing on its copy of `bar`
-__device__ __forceinline__ void st_async16(void* slot, uint64_t* bar, uint32_t rank, float x, float y, int z) {
+__device__ __forceinline__ void st_async16(void* slot, uint64_t* bar, uint32_t rank, uint32_t x, uint32_t y, int z) {
     uint32_t rs, rb;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rs) : "r"(smem_u32(slot)), "r"(rank));
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rb) : "r"(smem_u32(bar)), "r"(rank));
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(rs),
-                 "r"(__float_as_uint(x)), "r"(__float_as_uint(y)), "r"(z), "r"(0), "r"(rb)
+                 "r"(x), "r"(y), "r"(z), "r"(0), "r"(rb)
                  : "memory");
 }
 
@@ -329,11 +361,12 @@ __global__ void __launch_bounds__(kVsThreads) verify_cluster_kernel(const Verify
     const int T = a.T, N = a.N, V = a.V;
     __shared__ int s_tok[kVsMaxTree], s_par[kVsMaxTree], s_dep[kVsMaxTree], s_rk[kVsMaxTree];
     __shared__ int s_kids[kVsWarps][kVsMaxKids];  // each warp's list of a node's children
-    __shared__ __align__(16) float4 slots[2][kVsMaxCtas * kVsWarps];  // partial totals (h, l, last entry > 0) by exchange
+    // partial totals by exchange: a float pair's words, or a fixed-point sum's and the last entry > 0
+    __shared__ __align__(16) uint4 slots[2][kVsMaxCtas * kVsWarps];
     __shared__ __align__(8) uint64_t bar[2];
-    __shared__ FF seg[E * kVsWarps];  // the bonus draw: sums of 32 consecutive entries
-    __shared__ int s_seg, s_pick;
-    __shared__ double s_before;
+    __shared__ fx64 seg[E * kVsWarps];  // the bonus draw: sums of 32 consecutive entries
+    __shared__ int s_seg;
+    __shared__ fx64 s_before;
 
     if (t == 0) {
         mbar_init(&bar[0], 1);
@@ -348,21 +381,16 @@ __global__ void __launch_bounds__(kVsThreads) verify_cluster_kernel(const Verify
     }
     cluster_sync();  // (also a CTA barrier) every CTA's barriers are ready for remote arrivals
 
-    // Sends this warp's part to every CTA and waits for all of them: each warp then finds the
-    // partial of warp w of CTA j in its CTA's slots[x & 1][16 j + w]. Two sets of slots and barriers
+    // Sends this warp's part (the same in all lanes) to every CTA and waits for all of them: each
+    // warp then finds the partial of warp w of CTA j in its CTA's slots[x & 1][16 j + w]. Two sets of slots and barriers
     // alternate: exchange x + 2 reaches a CTA only after all of its warps, having read x, have
     // sent x + 1. False when the bounded wait ran out.
     int xch = 0;
     bool ok = true;
-    auto send = [&](FF part, int last) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            part = ff_add(part, ff_shfl_xor(part, o));
-            last = max(last, __shfl_xor_sync(0xffffffffu, last, o));
-        }
+    auto send = [&](uint32_t lo, uint32_t hi, int last) {
         const int p = xch & 1;
         if (t == 0) mbar_arrive_expect_tx(&bar[p], 16u * kVsWarps * (uint32_t)C);
-        if (lane < C) st_async16(&slots[p][c * kVsWarps + warp], &bar[p], (uint32_t)lane, part.h, part.l, last);
+        if (lane < C) st_async16(&slots[p][c * kVsWarps + warp], &bar[p], (uint32_t)lane, lo, hi, last);
         if (!mbar_try_wait_cluster(&bar[p], (uint32_t)(xch >> 1) & 1u)) {
             const uint64_t t0 = globaltimer_ns();
             while (!mbar_try_wait_cluster(&bar[p], (uint32_t)(xch >> 1) & 1u))
@@ -373,23 +401,6 @@ __global__ void __launch_bounds__(kVsThreads) verify_cluster_kernel(const Verify
         }
         ok = __all_sync(0xffffffffu, ok);
         ++xch;
-    };
-    // the sums of the CTAs' partials of the last exchange: lane 4 j holds CTA j's (j < C); 0 elsewhere
-    auto cta_totals = [&]() {
-        FF v;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int i = 4 * lane + u;
-            if (i < C * kVsWarps) {
-                const float4 x = slots[(xch - 1) & 1][i];
-                FF y;
-                y.h = x.x;
-                y.l = x.y;
-                v = ff_add(v, y);
-            }
-        }
-        v = ff_add(v, ff_shfl_xor(v, 1));
-        return ff_add(v, ff_shfl_xor(v, 2));
     };
 
     int cur = 0, n = 0;
@@ -446,8 +457,7 @@ __global__ void __launch_bounds__(kVsThreads) verify_cluster_kernel(const Verify
         const float ku = lane < m ? a.u_acc[(size_t)b * T + kid] : 0.f;
         __syncwarp();  // (s_kids is rewritten at the next node)
 
-        FF left;  // 1 - the q mass of the tokens drawn so far at this node
-        left.h = 1.f;
+        fx64 left = kFxOne;  // 1 - the q mass of the tokens drawn so far at this node
         float inv = 1.f;
         int next = -1;
         for (int i = 0; i < m; ++i) {
@@ -484,17 +494,30 @@ __global__ void __launch_bounds__(kVsThreads) verify_cluster_kernel(const Verify
                 ps[u].h = part[u].s;
                 ps[u].l = -part[u].c;
             }
-            send(ff_add(ff_add(ps[0], ps[1]), ff_add(ps[2], ps[3])), -1);
-            if (!ok) break;
-            FF Z = cta_totals();
+            FF Z = ff_add(ff_add(ps[0], ps[1]), ff_add(ps[2], ps[3]));
 #pragma unroll
-            for (int o = 4; o < 32; o <<= 1) Z = ff_add(Z, ff_shfl_xor(Z, o));
+            for (int o = 16; o > 0; o >>= 1) Z = ff_add(Z, ff_shfl_xor(Z, o));
+            const float drop = __shfl_sync(0xffffffffu, kq, i);
+            left = drop < 2.f ? left - min(left, fx(drop)) : 0ull;  // (no proposal: nothing is left)
+            inv = left ? fx_rcp(left) : 0.f;
+            send(__float_as_uint(Z.h), __float_as_uint(Z.l), -1);
+            if (!ok) break;
+            Z = FF{};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int j = 4 * lane + u;
+                if (j < C * kVsWarps) {
+                    const uint4 x = slots[(xch - 1) & 1][j];
+                    FF y;
+                    y.h = __uint_as_float(x.x);
+                    y.l = __uint_as_float(x.y);
+                    Z = ff_add(Z, y);
+                }
+            }
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) Z = ff_add(Z, ff_shfl_xor(Z, o));
             invZ = Z.h > 0.f ? ff_rcp(Z) : 0.f;
             from_p = false;
-            FF drop;
-            drop.h = -__shfl_sync(0xffffffffu, kq, i);
-            left = ff_add(left, drop);
-            inv = left.h > 0.f ? ff_rcp(left) : 0.f;
         }
         if (next < 0) break;  // every child rejected (or a malformed node)
         if (c == 0 && t == 0) a.path[(size_t)b * N + n] = next;
@@ -507,52 +530,51 @@ __global__ void __launch_bounds__(kVsThreads) verify_cluster_kernel(const Verify
 
     // ---- the bonus token: inverse CDF of r. The CTAs' totals name the CTA that holds it, the
     // sums of its 32-entry segments the segment, a warp scan the entry.
-    const double u = a.u_bonus[(size_t)b * T + cur];
-    KahanF part[4];
+    const float uf = a.u_bonus[(size_t)b * T + cur];
+    const fx64 u = uf < 2.f ? fx(uf) : ~0ull;  // (u < a sum exactly when the deviate is below it)
+    fx64 mass = 0;
+    float about = 0.f;
     int last = -1;
 #pragma unroll
     for (int e = 0; e < E; ++e) {
         if (!from_p) w[e] = __fmul_rn(w[e], invZ);
-        part[e & 3].add(w[e]);
+        mass += fx(w[e]);
+        about += fx_clamp(w[e]);
         if (w[e] > 0.f) last = c * S + e * kVsThreads + t;
     }
-    FF ps[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        ps[k].h = part[k].s;
-        ps[k].l = -part[k].c;
-    }
-    int owner = -1, c_last = -1, all_last = -1;
-    double prefix = 0.0;  // the total of the CTAs before this one
+    if (about >= 3.f) mass = ~0ull;  // (may have wrapped at 4; no deviate is between)
+    int owner = -1, all_last = -1;
+    fx64 prefix = 0;  // the total of the CTAs before this one
     if (ok) {
-        send(ff_add(ff_add(ps[0], ps[1]), ff_add(ps[2], ps[3])), last);
-        FF run = cta_totals();  // inclusive over CTAs: lane 4 j
-#pragma unroll
-        for (int o = 4; o < 32; o <<= 1) {
-            FF up;
-            up.h = __shfl_up_sync(0xffffffffu, run.h, o);
-            up.l = __shfl_up_sync(0xffffffffu, run.l, o);
-            if (lane >= o) run = ff_add(up, run);
-        }
-        const bool pass = u < ff_value(run);
-        const unsigned hit = __ballot_sync(0xffffffffu, pass && lane % 4 == 0 && lane / 4 < C);
-        owner = hit ? (__ffs(hit) - 1) / 4 : -1;
-        if (c > 0) {
-            FF bf;
-            bf.h = __shfl_sync(0xffffffffu, run.h, 4 * c - 4);
-            bf.l = __shfl_sync(0xffffffffu, run.l, 4 * c - 4);
-            prefix = ff_value(bf);
-        }
-        for (int i = lane; i < C * kVsWarps; i += 32) {
-            const int l = __float_as_int(slots[(xch - 1) & 1][i].z);
-            all_last = max(all_last, l);
-            if (i / kVsWarps == c) c_last = max(c_last, l);
-        }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-            all_last = max(all_last, __shfl_xor_sync(0xffffffffu, all_last, o));
-            c_last = max(c_last, __shfl_xor_sync(0xffffffffu, c_last, o));
+            mass = fx_add(mass, __shfl_xor_sync(0xffffffffu, mass, o));
+            last = max(last, __shfl_xor_sync(0xffffffffu, last, o));
         }
+        send((uint32_t)mass, (uint32_t)(mass >> 32), last);
+        fx64 run = 0;  // inclusive over CTAs: lanes 4 j .. 4 j + 3
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int i = 4 * lane + k;
+            if (i < C * kVsWarps) {
+                const uint4 x = slots[(xch - 1) & 1][i];
+                run = fx_add(run, (fx64)x.y << 32 | x.x);
+                all_last = max(all_last, (int)x.z);
+            }
+        }
+        run = fx_add(run, __shfl_xor_sync(0xffffffffu, run, 1));
+        run = fx_add(run, __shfl_xor_sync(0xffffffffu, run, 2));
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) {
+            const fx64 up = __shfl_up_sync(0xffffffffu, run, o);
+            if (lane >= o) run = fx_add(up, run);
+        }
+        const unsigned hit = __ballot_sync(0xffffffffu, u < run && lane % 4 == 0 && lane / 4 < C);
+        owner = hit ? (__ffs(hit) - 1) / 4 : -1;
+        prefix = __shfl_sync(0xffffffffu, run, max(4 * c - 4, 0));
+        if (c == 0) prefix = 0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) all_last = max(all_last, __shfl_xor_sync(0xffffffffu, all_last, o));
     }
     if (!ok && t == 0) atomicOr(a.status, ST_TIMEOUT);
     for (int i = n + t; i < N && c == 0; i += kVsThreads) a.path[(size_t)b * N + i] = -1;
@@ -560,71 +582,61 @@ __global__ void __launch_bounds__(kVsThreads) verify_cluster_kernel(const Verify
         a.n_accept[b] = n;
         if (!ok || owner < 0) a.bonus[b] = max(all_last, 0);
     }
-    if (!__syncthreads_or(!ok) && owner == c) {
-        FF v[E];
+    if (!__syncthreads_or(!ok) && owner == c) {  // (one segment, and one entry of it, passes u)
+        // the transposing reduction's first step forms the units again, two by two: held since
+        // above they would spill
+        fx64 v[E / 2];
 #pragma unroll
-        for (int e = 0; e < E; ++e) v[e].h = w[e];
-        ff_multi_sum<E, 16>(v, lane);
+        for (int e = 0; e < E / 2; ++e) {
+            asm volatile("" : "+f"(w[e]), "+f"(w[e + E / 2]));
+            const fx64 x = fx(w[e]), y = fx(w[e + E / 2]);
+            v[e] = fx_add(lane & 16 ? y : x, __shfl_xor_sync(0xffffffffu, lane & 16 ? x : y, 16));
+        }
+        fx_multi_sum<E / 2, 8>(v, lane);
         constexpr int LG = 32 / E;  // lanes that hold the same sum
         if (lane % LG == 0) seg[(lane / LG) * kVsWarps + warp] = v[0];
-        if (t == 0) {
-            s_seg = -1;
-            s_pick = INT_MAX;
-        }
         __syncthreads();
         if (warp == 0) {  // lane l scans segments [l E / 2, (l + 1) E / 2)
             constexpr int PL = E * kVsWarps / 32;
-            FF sum;
+            fx64 sum = 0;
 #pragma unroll
-            for (int j = 0; j < PL; ++j) sum = ff_add(sum, seg[lane * PL + j]);
-            FF inc = sum;
+            for (int j = 0; j < PL; ++j) sum = fx_add(sum, seg[lane * PL + j]);
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                FF up;
-                up.h = __shfl_up_sync(0xffffffffu, inc.h, o);
-                up.l = __shfl_up_sync(0xffffffffu, inc.l, o);
-                if (lane >= o) inc = ff_add(up, inc);
+                const fx64 up = __shfl_up_sync(0xffffffffu, sum, o);
+                if (lane >= o) sum = fx_add(up, sum);
             }
-            const unsigned hit = __ballot_sync(0xffffffffu, u < prefix + ff_value(inc));
-            FF ex;
-            ex.h = __shfl_up_sync(0xffffffffu, inc.h, 1);
-            ex.l = __shfl_up_sync(0xffffffffu, inc.l, 1);
+            const fx64 inc = fx_add(prefix, sum);
+            const fx64 before = __shfl_up_sync(0xffffffffu, inc, 1);
+            const unsigned hit = __ballot_sync(0xffffffffu, u < inc);
             if (hit && lane == __ffs(hit) - 1) {
-                FF run = lane ? ex : FF{};
-                int found = lane * PL + PL - 1;
-                for (int j = 0; j < PL; ++j) {
-                    const FF nx = ff_add(run, seg[lane * PL + j]);
-                    if (u < prefix + ff_value(nx)) {
-                        found = lane * PL + j;
-                        break;
-                    }
-                    if (j + 1 < PL) run = nx;
+                fx64 run = lane ? before : prefix;
+                int j = 0;
+                for (; j + 1 < PL; ++j) {
+                    const fx64 nx = fx_add(run, seg[lane * PL + j]);
+                    if (u < nx) break;
+                    run = nx;
                 }
-                s_seg = found;
-                s_before = prefix + ff_value(run);
+                s_seg = lane * PL + j;
+                s_before = run;
             }
         }
         __syncthreads();
-        if (s_seg >= 0 && warp == s_seg % kVsWarps) {
+        if (warp == s_seg % kVsWarps) {
             const int es = s_seg / kVsWarps;
-            FF inc;
+            float mine = 0.f;
 #pragma unroll
             for (int e = 0; e < E; ++e)
-                if (e == es) inc.h = w[e];
+                if (e == es) mine = w[e];
+            fx64 inc = fx_add(lane == 0 ? s_before : 0ull, fx(mine));
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                FF up;
-                up.h = __shfl_up_sync(0xffffffffu, inc.h, o);
-                up.l = __shfl_up_sync(0xffffffffu, inc.l, o);
-                if (lane >= o) inc = ff_add(up, inc);
+                const fx64 up = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc = fx_add(up, inc);
             }
-            const unsigned hit = __ballot_sync(0xffffffffu, u < s_before + ff_value(inc));
-            if (hit && lane == 0) s_pick = c * S + es * kVsThreads + warp * 32 + __ffs(hit) - 1;
+            const unsigned hit = __ballot_sync(0xffffffffu, u < inc);
+            if (hit && lane == 0) a.bonus[b] = c * S + es * kVsThreads + warp * 32 + __ffs(hit) - 1;
         }
-        __syncthreads();
-        // (no entry passes u only when the sums' last bits differ at a segment's end: then the
-        // last entry of this CTA with r > 0)
-        if (t == 0) a.bonus[b] = s_pick != INT_MAX ? s_pick : max(c_last, 0);
     }
     cluster_sync();  // no CTA leaves while another may still write its shared memory
 }
