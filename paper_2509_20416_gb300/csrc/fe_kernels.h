@@ -280,7 +280,6 @@ struct LmHeadView {
     const void* final_norm;  // [d]
     bool mma;
     bool pdl;
-    int lm_16row;  // fe_handle's choice of the head up to 16 rows (1 / 0 forced, -1 by rule)
     fe_dtype dtype;
     int d, V, N, max_batch, top_k_max, n_slabs;
     float eps;

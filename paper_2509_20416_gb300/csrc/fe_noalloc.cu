@@ -135,11 +135,10 @@ extern "C" FE_API fe_status fe_lm_head_topk_noalloc(fe_handle* h, const float* h
     lm.pdl = v.pdl;
     lm.first_full = true;  // (whatever precedes the call on the stream)
     uint16_t* operand = (uint16_t*)(base + kPartIdBytes + kPartValBytes + kPartMsBytes);
-    // the same choice of kernel as in a draft; the wide one's operand (32 rows) fits the array's
-    const bool wide = v.mma && (v.lm_16row == 0 ? lmhead_wide_ok(lm) : v.lm_16row < 0 && lmhead_wide_small(lm, v.dev));
-    if (wide) lm.n_slabs = lmhead_wide_slabs(v.V, v.dev);
-    const cudaError_t e = wide    ? launch_lmhead_wide(lm, operand, v.dev, st)
-                          : v.mma ? launch_lmhead_mma(lm, operand, v.dev, st)
-                                  : launch_lmhead(v.dtype, lm, v.dev, st);
+    // Always the 16-row kernel on the tensor cores, also where a draft takes the wide one: the wide
+    // kernel's base-2 statistics round logit * log2(e) / T once more, and its lse is up to 1.2 times
+    // as far from 64 bits (1.16e-6 against 1.00e-6 rms over 16 rows of 90111 entries; 4.6e-6
+    // against 4.4e-6 over 128256).
+    const cudaError_t e = v.mma ? launch_lmhead_mma(lm, operand, v.dev, st) : launch_lmhead(v.dtype, lm, v.dev, st);
     return e == cudaSuccess ? FE_OK : FE_ERR_CUDA;
 }

@@ -809,7 +809,6 @@ bool fe::handle_lmhead_view(const fe_handle* h, LmHeadView* v) {
     v->final_norm = h->final_norm;
     v->mma = h->lm_mma;
     v->pdl = h->use_pdl;
-    v->lm_16row = h->lm_16row;
     v->dtype = h->cfg.dtype;
     v->d = h->cfg.d;
     v->V = h->cfg.vocab;
