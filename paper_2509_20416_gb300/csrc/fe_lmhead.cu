@@ -504,7 +504,7 @@ __device__ __forceinline__ bool merge_row(const LmHeadArgs& a, int zr, MergeScra
     if (t < ns) {
         int r = 0;
         for (int j = 0; j < ns; ++j) r += sc.first[j] > v[0] || (sc.first[j] == v[0] && j < t);
-        if (r == k - 1) sc.tau = v[0];
+        if (r == k - 1 && v[0] == v[0]) sc.tau = v[0];  // (a NaN compares above nothing: no threshold)
     }
     __syncthreads();
     const float tau = sc.tau;
