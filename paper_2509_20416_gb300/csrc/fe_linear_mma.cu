@@ -94,21 +94,56 @@ __device__ __forceinline__ float sumsq8(const float (&v)[8]) {
     return s;
 }
 
+// Takes x's largest bf16 part out of it.
+__device__ __forceinline__ uint32_t take_bf16(float& x) {
+    const uint32_t h = f32_to_bf16(x);
+    x -= bf16_to_f32((uint16_t)h);
+    return h;
+}
+
+// The same for any x: a finite one keeps a finite part, also where it would round to infinity; an
+// infinity or a NaN stays one and leaves 0.
+__device__ __forceinline__ uint32_t take_bf16_any(float& x) {
+    if (!(fabsf(x) < INFINITY)) {
+        const uint32_t h = x == x ? __float_as_uint(x) >> 16 : 0x7fffu;
+        x = 0.f;
+        return h;
+    }
+    uint32_t h = f32_to_bf16(x);
+    if ((h & 0x7fffu) == 0x7f80u) --h;
+    x -= bf16_to_f32((uint16_t)h);
+    return h;
+}
+
 // the bf16 operand chunk c of row b from 8 values: x = hi + lo (two splits) or hi + mid + lo,
-// split q in row q * B_pad + b
+// split q in row q * B_pad + b. Three splits stand in for a float32 product, which keeps
+// infinities and NaN apart from finite values: a chunk that holds one, or a value that rounds to
+// infinity (2^127 (2 - 2^-8) and above), is split by take_bf16_any.
 template <int NS>
 __device__ __forceinline__ void put_operand(uint16_t* xb, int N, int B_pad, int b, int c, const float (&v)[8]) {
     uint32_t w[NS][4];
+    float x[8];
+    uint32_t h[8], big = 0;
 #pragma unroll
-    for (int e = 0; e < 8; e += 2) {
-        float x0 = v[e], x1 = v[e + 1];
+    for (int e = 0; e < 8; ++e) {
+        x[e] = v[e];
+        big = max(big, __float_as_uint(v[e]) & 0x7fffffffu);
+    }
+    if (NS == 3 && big >= 0x7f7f8000u) {
 #pragma unroll
-        for (int q = 0; q < NS; ++q) {
-            const uint16_t h0 = f32_to_bf16(x0), h1 = f32_to_bf16(x1);
-            w[q][e / 2] = (uint32_t)h0 | ((uint32_t)h1 << 16);
-            x0 -= bf16_to_f32(h0);
-            x1 -= bf16_to_f32(h1);
+        for (int e = 0; e < 8; ++e) h[e] = take_bf16_any(x[e]);
+    } else {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) h[e] = take_bf16(x[e]);
+    }
+#pragma unroll
+    for (int q = 0; q < NS; ++q) {
+        if (q > 0) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) h[e] = take_bf16(x[e]);
         }
+#pragma unroll
+        for (int e = 0; e < 8; e += 2) w[q][e / 2] = h[e] | h[e + 1] << 16;
     }
     unsigned char* blk = (unsigned char*)xb + (size_t)(c / 8) * N * 128;
 #pragma unroll
@@ -615,6 +650,7 @@ __global__ void __launch_bounds__(lin_threads(NS), 1) linear_mma_kernel(const Li
                 }
                 tc_fence_after();
                 const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(buf * MT * N);
+                float big = 0.f;  // the largest compensated sum
 #pragma unroll 1
                 for (int h = 0; h < MT; ++h)
 #pragma unroll
@@ -638,6 +674,7 @@ __global__ void __launch_bounds__(lin_threads(NS), 1) linear_mma_kernel(const Li
                                 const float x0 = y - vc[b + i], s0 = v[b + i] + x0;
                                 vc[b + i] = (s0 - v[b + i]) - x0;
                                 v[b + i] = s0;
+                                big = fmaxf(big, fabsf(s0));
                             }
                         }
                     }
@@ -646,6 +683,13 @@ __global__ void __launch_bounds__(lin_threads(NS), 1) linear_mma_kernel(const Li
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&st.tempty[buf]);
+                if constexpr (TM)
+                    if (big == INFINITY) {  // an infinite sum has lost nothing: left alone, the next
+                                            // addition would be inf - inf
+#pragma unroll
+                        for (int b = 0; b < W; ++b)
+                            if (fabsf(v[b]) == INFINITY) vc[b] = 0.f;
+                    }
                 if (++buf == NA) { buf = 0; pt ^= 1u; }
             }
             if (!ok) break;
