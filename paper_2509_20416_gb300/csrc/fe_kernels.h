@@ -185,7 +185,8 @@ bool linear_mma_ok(int M, int K, int B);
 size_t linear_mma_xb_bytes(int K, int B, int splits);
 cudaError_t linear_mma_map(const void* W, int M, int K, CUtensorMap* map);
 size_t linear_mma_part_bytes(int B, const DeviceInfo& dev);
-int linear_mma_mt(int M, int B, int splits);  // 128-row tiles to a unit of B rows' product
+// 128-row tiles to a unit of B rows' product
+int linear_mma_mt(int M, int B, int splits, const DeviceInfo& dev);
 int linear_mma_grid(int M, int K, const DeviceInfo& dev, int mt);
 cudaError_t linear_mma_prepare(const DeviceInfo& dev);
 // the completion-counter buffer: the last norm_post phase's per-row scales and its prep's

@@ -20,7 +20,7 @@
 //     buffers), warps 0-3 read TMEM (thread = output row) and add hi + lo.
 //   - Two forms (LinearArgs::splits). Handles of 9..32 sequences: their own weight layout (one
 //     contiguous 16 KB copy per unit), two splits, one accumulation chain per tile (commit blocks
-//     of up to 128 rows: kPairTiles). Handles of up to 8 and of 33..64 sequences (drafts of 2 to
+//     of up to 128 rows: linear_mma_mt). Handles of up to 8 and of 33..64 sequences (drafts of 2 to
 //     16 hidden rows and commits, where linear_tc_us is below linear_stream_us): the streaming
 //     kernel's tile layout, which a tensor map reads as the same operand, so that a
 //     handle needs one copy of its weights for both kernels; THREE splits (hi + mid + lo are
@@ -55,15 +55,6 @@ constexpr int kLinMaxAccs = 8;
 __host__ __device__ constexpr int acc_buffers(int N, int ns, int mt) {
     return ns == 3 ? (512 / N < kLinMaxAccs ? 512 / N : kLinMaxAccs) : mt == 2 ? 1 : 2;
 }
-
-// 128-row tiles to a unit. Above 64 rows and with more tiles than CTAs a unit is a 64-column
-// block of TWO tiles sharing one operand block: with one tile the operand (32 KB a block at 128
-// rows, two splits) makes an SM read 48 KB from L2 per 16 KB of weights, and gate/up of the 8B
-// shape (28672 x 4096) took 64 us; with two 48 (a commit of 150 rows: 1289 -> 1215 us). Their
-// accumulators of up to 512 columns fill the tensor memory (no second buffer), and a pair is cut
-// between twice as many CTAs: matrices of few tiles lose (O projection 15 -> 19 us, W_fuse
-// 26 -> 31).
-constexpr int kPairTiles = 152;
 
 // operand rows (MMA columns): the splits' blocks of B_pad rows, to a multiple of 16
 __host__ __device__ constexpr int operand_rows(int bpad, int ns) { return (ns * bpad + 15) / 16 * 16; }
@@ -737,7 +728,15 @@ __global__ void __launch_bounds__(lin_threads(NS), 1) linear_mma_kernel(const Li
 }
 
 // ---- host side -----------------------------------------------------------------------------
-int linear_mma_mt(int M, int B, int splits) { return splits == 2 && B > kTileMaxRows && (M + 127) / 128 > kPairTiles ? 2 : 1; }
+// Above 64 rows and with more tiles than CTAs a unit is a 64-column block of TWO tiles sharing one
+// operand block: with one tile the operand (32 KB a block at 128 rows, two splits) makes an SM read
+// 48 KB from L2 per 16 KB of weights, and gate/up of the 8B shape (28672 x 4096, 224 tiles on 152
+// SMs) took 64 us; with two 48 (a commit of 150 rows: 1289 -> 1215 us). Their accumulators of up to
+// 512 columns fill the tensor memory (no second buffer), and a pair is cut between twice as many
+// CTAs: matrices of few tiles lose (O projection 15 -> 19 us, W_fuse 26 -> 31).
+int linear_mma_mt(int M, int B, int splits, const DeviceInfo& dev) {
+    return splits == 2 && B > kTileMaxRows && (M + 127) / 128 > dev.num_sms ? 2 : 1;
+}
 
 namespace {
 
@@ -788,7 +787,7 @@ cudaError_t launch_product(const LinearArgs& a, uint16_t* xb, float* part, int* 
     if constexpr (BP <= kTileMaxRows)
         if (a.splits == 3) return launch_bp<BP, 3>(a, xb, part, counters, aux, dev, st, grid);
     if constexpr (BP > kTileMaxRows)
-        if (linear_mma_mt(a.M, a.B, a.splits) == 2) return launch_bp<BP, 2, 2>(a, xb, part, counters, aux, dev, st, grid);
+        if (linear_mma_mt(a.M, a.B, a.splits, dev) == 2) return launch_bp<BP, 2, 2>(a, xb, part, counters, aux, dev, st, grid);
     return launch_bp<BP, 2>(a, xb, part, counters, aux, dev, st, grid);
 }
 
@@ -858,7 +857,7 @@ cudaError_t launch_linear_mma(const LinearArgs& a, uint16_t* xb, float* part, in
     const int BP = linear_mma_bpad(a.B);
     unsigned char* aux = (unsigned char*)counters;
     int* tctr = (int*)(aux + tile_counter_offset(dev));
-    const int grid = linear_mma_grid(a.M, a.K, dev, linear_mma_mt(a.M, a.B, a.splits));
+    const int grid = linear_mma_grid(a.M, a.K, dev, linear_mma_mt(a.M, a.B, a.splits, dev));
     // finish + normalise a row per CTA (only when the scale goes on the operand)
     const bool row_cta = !a.norm_post && a.prev.active && a.pro == PRO_RMSNORM;
     if (row_cta && ((size_t)a.K * sizeof(float) > kXprepRowSmem || a.prev.epi == EPI_SWIGLU || a.splits != 2))

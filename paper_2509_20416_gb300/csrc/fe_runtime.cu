@@ -386,7 +386,7 @@ fe_status enqueue_forward(fe_handle* h, const fe_forward_args* a, cudaStream_t s
                 pending.part = h->lin_part;
                 pending.M = L.M;
                 pending.K = L.K;
-                pending.mt = linear_mma_mt(L.M, L.B, L.splits);
+                pending.mt = linear_mma_mt(L.M, L.B, L.splits, h->dev);
                 pending.G = linear_mma_grid(L.M, L.K, h->dev, pending.mt);
                 pending.epi = L.epi;
                 pending.y = L.y;
@@ -678,7 +678,7 @@ fe_status enqueue_commit_rows(fe_handle* h, const fe_commit_args* a, cudaStream_
         if (L.defer) {
             pending.active = 1;
             pending.part = h->lin_part;
-            pending.M = L.M; pending.K = L.K; pending.mt = linear_mma_mt(L.M, L.B, L.splits);
+            pending.M = L.M; pending.K = L.K; pending.mt = linear_mma_mt(L.M, L.B, L.splits, h->dev);
             pending.G = linear_mma_grid(L.M, L.K, h->dev, pending.mt);
             pending.epi = L.epi; pending.y = L.y; pending.ldy = L.ldy; pending.y2 = L.y2; pending.ldy2 = L.ldy2;
             pending.ybase = L.ybase;
