@@ -304,7 +304,8 @@ FE_API fe_status fe_verify_greedy(fe_handle *h, int32_t B, int32_t top_k, const 
  *  n_accept  device [B] int32; bonus device [B] int32
  * Asynchronous on `stream`; FE_ERR_INVALID_ARG for bad host-side arguments; a token or depth
  * out of range in the tree ends that sequence's walk and sets FE_ERR_DEVICE in the status
- * word. The handle holds one V-float residual buffer per sequence for it. */
+ * word. For vocabularies above 131072 entries the handle holds one V-float residual buffer per
+ * sequence for it. */
 FE_API fe_status fe_verify_sampled(fe_handle *h, int32_t B, int32_t top_k, const fe_tree *tree,
                                    const int32_t *topk_rank, const float *q, const float *p, const float *u_acc,
                                    const float *u_bonus, int32_t *path, int32_t *n_accept, int32_t *bonus,

@@ -367,6 +367,9 @@ cudaError_t launch_verify(int B, int T, int max_path, const int* prefix_len, con
                           const int* depth, const int* target_next, int* pos, int* path, int* n_accept, int* bonus,
                           cudaStream_t st);
 // lossless verification of a sampled tree (fe_verify.cu): one CTA per sequence
+// vocabularies up to here are verified from registers; beyond, the residual needs rbuf
+constexpr int kVerifyMaxRegV = 131072;
+
 struct VerifySampledArgs {
     int T, N, V;
     const int *tok, *parent, *depth;  // [B, T] trees in fe_build_tree's layout
@@ -374,7 +377,7 @@ struct VerifySampledArgs {
     const float* q;                   // [B, N, V] the drafter's proposal per depth
     const float* p;                   // [B, T, V] the target's distribution after each node
     const float *u_acc, *u_bonus;     // [B, T]
-    float* rbuf;                      // [B, V] scratch: each sequence's residual
+    float* rbuf;                      // [B, V] scratch: each sequence's residual (V > kVerifyMaxRegV)
     int *path, *n_accept, *bonus;     // [B, N], [B], [B]
     int* status;
 };

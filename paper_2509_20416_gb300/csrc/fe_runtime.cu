@@ -109,7 +109,7 @@ struct fe_handle {
     const void *w_fuse = nullptr, *w_in = nullptr, *embed = nullptr, *lm_head = nullptr, *final_norm = nullptr;
     std::vector<LayerPacked> layers;
     float* rope_cs = nullptr;
-    void* cfeat = nullptr;  // commit: one block's gathered feature rows [<= 32, 3d]
+    void* cfeat = nullptr;  // commit: one block's gathered feature rows [<= commit_block_rows, 3d]
     int* ctok = nullptr;    // commit: their tokens
     // commit by rows (null where that path does not serve the handle): the plan, and the
     // attention partials of a block's rows
@@ -123,7 +123,8 @@ struct fe_handle {
     float *lm_part_val = nullptr, *lm_part_ms = nullptr;
     float* lm_part_lg = nullptr;  // sampling: the logits of the partials' candidates
     void* loss_part = nullptr;    // fe_draft_loss: its vocabulary chunks' sums
-    float* vs_rbuf = nullptr;     // fe_verify_sampled: each sequence's residual distribution [max_batch, V]
+    // fe_verify_sampled: each sequence's residual distribution [max_batch, V] (null up to kVerifyMaxRegV)
+    float* vs_rbuf = nullptr;
     int* status = nullptr;
     int* attn_counters = nullptr;
     bool lm_mma = false;      // LM head packed for (and run on) the tensor cores
@@ -1082,7 +1083,7 @@ fe_status fe_draft_init(const fe_config* cfg, const fe_weights* w, void* stream,
             h->lm_mma ? lmhead_mma_split_bytes(16, h->dev) : 0,                // LM head: split-tile parts
             h->lm_mma ? (size_t)h->dev.num_sms * sizeof(int) : 0,             // ... and their flags
             R * h->lm_slabs * k * 4,                                          // LM-head partial logits (sampling)
-            B * (size_t)c.vocab * 4,                                          // sampled verification's residuals
+            c.vocab > kVerifyMaxRegV ? B * (size_t)c.vocab * 4 : 0,           // sampled verification's residuals
             cm ? (B + 1) * sizeof(int) : 0, cm ? sizeof(int) : 0,             // commit plan: off, total
             cm ? crows * sizeof(int) : 0, cm ? crows * sizeof(int) : 0,       // ... x_row, nact
             cm ? (size_t)Rmma * H * h->attn_nsplit * (hd + 4) * 4 : 0,        // ... attention partials
@@ -1115,7 +1116,7 @@ fe_status fe_draft_init(const fe_config* cfg, const fe_weights* w, void* stream,
         h->lm_split_part = h->lm_mma ? (float*)(s + off[22]) : nullptr;
         h->lm_split_flag = h->lm_mma ? (int*)(s + off[23]) : nullptr;
         h->lm_part_lg = (float*)(s + off[24]);
-        h->vs_rbuf = (float*)(s + off[25]);
+        h->vs_rbuf = c.vocab > kVerifyMaxRegV ? (float*)(s + off[25]) : nullptr;
         h->loss_part = s + off[32];
         h->rows_x = h->lin_tile && B > 1 ? (float*)(s + off[31]) : nullptr;
         if (cm) {

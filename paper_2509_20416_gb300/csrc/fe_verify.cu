@@ -662,13 +662,14 @@ cudaError_t launch_cluster(const VerifySampledArgs& a, int B, int C, cudaStream_
 
 cudaError_t launch_verify_sampled(const VerifySampledArgs& a, int B, cudaStream_t st) {
     // entries per thread by the vocabulary: a small one stays in one CTA (no exchange across
-    // CTAs), larger ones take 8; beyond 8 x 512 x 32 entries the registers no longer hold it
-    if (a.T <= kVsMaxTree) {
-        if (a.V <= 8 * kVsThreads) return launch_cluster<8>(a, B, 1, st);
-        if (a.V <= kVsMaxCtas * kVsThreads * 8) return launch_cluster<8>(a, B, kVsMaxCtas, st);
-        if (a.V <= kVsMaxCtas * kVsThreads * 16) return launch_cluster<16>(a, B, kVsMaxCtas, st);
-        if (a.V <= kVsMaxCtas * kVsThreads * 32) return launch_cluster<32>(a, B, kVsMaxCtas, st);
-    }
+    // CTAs), larger ones take 8; beyond 8 x 512 x 32 entries the registers no longer hold it.
+    // (A handle's trees have at most kVsMaxTree nodes.)
+    static_assert(kVerifyMaxRegV == kVsMaxCtas * kVsThreads * 32);
+    if (a.V <= 8 * kVsThreads) return launch_cluster<8>(a, B, 1, st);
+    if (a.V <= kVsMaxCtas * kVsThreads * 8) return launch_cluster<8>(a, B, kVsMaxCtas, st);
+    if (a.V <= kVsMaxCtas * kVsThreads * 16) return launch_cluster<16>(a, B, kVsMaxCtas, st);
+    if (a.V <= kVerifyMaxRegV) return launch_cluster<32>(a, B, kVsMaxCtas, st);
+    if (!a.rbuf) return cudaErrorInvalidValue;
     verify_sampled_kernel<<<B, kVsThreads, 0, st>>>(a);
     return cudaGetLastError();
 }
