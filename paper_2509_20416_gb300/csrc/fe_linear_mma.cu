@@ -61,8 +61,9 @@ __host__ __device__ constexpr int operand_rows(int bpad, int ns) { return (ns * 
 
 struct LinMmaState {
     uint64_t full[kLinMaxStages], empty[kLinMaxStages], tfull[kLinMaxAccs], tempty[kLinMaxAccs];
+    uint64_t drain[2];  // the MMA issuers', should a wait give up
     uint32_t tmem_base;
-    int abort;
+    int abort, issued;  // issued: copies the producer asked for
 };
 
 }  // namespace
@@ -449,6 +450,8 @@ __global__ void __launch_bounds__(lin_threads(NS), 1) linear_mma_kernel(const Li
             mbar_init(&st.tfull[i], 1);
             mbar_init(&st.tempty[i], 4);
         }
+        mbar_init(&st.drain[0], 1);
+        mbar_init(&st.drain[1], 1);
         st.abort = 0;
         mbar_fence_init();
     }
@@ -502,7 +505,8 @@ __global__ void __launch_bounds__(lin_threads(NS), 1) linear_mma_kernel(const Li
             // (it - S) / S of empty[slot]
             int slot = 0, acc = 0;
             uint32_t pe = 0, pa = 0;
-            for (int it = pre; it < total; ++it) {
+            int it = pre;
+            for (; it < total; ++it) {
                 if (!mbar_wait_abortable(one_commit ? &st.tfull[acc] : &st.empty[slot], one_commit ? pa : pe, a.status,
                                          &st.abort))
                     break;
@@ -514,6 +518,7 @@ __global__ void __launch_bounds__(lin_threads(NS), 1) linear_mma_kernel(const Li
                 if (++kx == nkb) kx = 0;
                 if (++slot == S) { slot = 0; pe ^= 1u; }
             }
+            st.issued = it;
         }
     } else if (TM && warp >= 5) {  // ---- MMA issuers: warps 5 and 6 take alternate units
         // (one thread needs ~850 cycles for a unit's waits, four MMAs and commits, more than
@@ -538,6 +543,7 @@ __global__ void __launch_bounds__(lin_threads(NS), 1) linear_mma_kernel(const Li
                 if ((slot += 2) >= S) { slot -= S; pf ^= 1u; }
                 if ((buf += 2) >= NA) { buf -= NA; pe ^= 1u; }
             }
+            if (*(volatile int*)&st.abort) drain_mmas(&st.drain[warp - 5], a.status);
         }
     } else if (warp == 5) {  // ---- MMA issuer
         if (lane == 0) {
@@ -572,6 +578,7 @@ __global__ void __launch_bounds__(lin_threads(NS), 1) linear_mma_kernel(const Li
                 }
                 if (ok) tc_commit(&st.tfull[buf]);
             }
+            if (*(volatile int*)&st.abort) drain_mmas(&st.drain[0], a.status);
         }
     } else {  // ---- epilogue warps 0..3: TMEM lane 32 w + l = output row of the tile
         // rs_s: the per-row factor of the products (norm_post: the RMSNorm scales, else 1)
@@ -724,6 +731,7 @@ __global__ void __launch_bounds__(lin_threads(NS), 1) linear_mma_kernel(const Li
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (t == 0 && *(volatile int*)&st.abort) drain_copies(st.full, S, st.issued, a.status);
     if (warp == 0) tc_dealloc(tmem, tmem_cols);
 }
 

@@ -724,9 +724,9 @@ __device__ __forceinline__ int ld_acquire_gpu(const int* p) {
 }
 
 struct MmaState {
-    uint64_t full[kMmaMaxStages], empty[kMmaMaxStages], tfull[2], tempty[2], ebar;
+    uint64_t full[kMmaMaxStages], empty[kMmaMaxStages], tfull[2], tempty[2], ebar, drain;
     uint32_t tmem_base;
-    int last, abort;
+    int abort, issued;  // issued: copies the producer asked for
 };
 
 __global__ void __launch_bounds__(kMmaThreads, 1) lmhead_mma_kernel(const LmHeadArgs a, const uint16_t* zb, int R_pad,
@@ -770,6 +770,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) lmhead_mma_kernel(const LmHead
             mbar_init(&st.tempty[i], 4);
         }
         mbar_init(&st.ebar, 4);  // the four epilogue warps (split-tile hand-offs)
+        mbar_init(&st.drain, 1);
         st.abort = 0;
         mbar_fence_init();
     }
@@ -805,7 +806,8 @@ __global__ void __launch_bounds__(kMmaThreads, 1) lmhead_mma_kernel(const LmHead
             // (it - S) / S of empty[slot]
             int slot = 0;
             uint32_t pe = 0;
-            for (int it = pre; it < total; ++it) {
+            int it = pre;
+            for (; it < total; ++it) {
                 if (!mbar_wait_abortable(&st.empty[slot], pe, a.status, &st.abort)) break;
                 unsigned char* dst = ring + (size_t)slot * stage_bytes;
                 mbar_arrive_expect_tx(&st.full[slot], 16384u + (uint32_t)N * 128u);
@@ -815,6 +817,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) lmhead_mma_kernel(const LmHead
                 if (++kb == nkb) kb = 0;
                 if (++slot == S) { slot = 0; pe ^= 1u; }
             }
+            st.issued = it;
         }
     } else if (warp == 5) {  // ---- MMA issuer
         if (lane == 0) {
@@ -846,6 +849,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) lmhead_mma_kernel(const LmHead
                 if (!ok) break;
                 tc_commit(&st.tfull[buf]);
             }
+            if (*(volatile int*)&st.abort) drain_mmas(&st.drain, a.status);
         }
     } else {  // ---- epilogue warps 0..3: TMEM lanes 32 w .. 32 w + 31 = vocabulary rows of the tile
         const int tr = warp * 32 + lane;  // row of the tile
@@ -919,6 +923,10 @@ __global__ void __launch_bounds__(kMmaThreads, 1) lmhead_mma_kernel(const LmHead
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (*(volatile int*)&st.abort) {  // (the ring is about to be written)
+        if (t == 0) drain_copies(st.full, S, st.issued, a.status);
+        __syncthreads();
+    }
     if (warp == 0) tc_dealloc(tmem, tmem_cols);
 
     // ---- this slab's partial per row (warp w: rows w, w + 6, ..): statistics and top-k;
@@ -1115,9 +1123,9 @@ constexpr int kWideThreads = 10 * 32;  // 8 epilogue warps, 1 producer warp, 1 M
 
 struct WideState {
     uint64_t wfull[kWideMaxW], zfull[kWideMaxW], done[kWideMaxW], tfull[2], tempty[2],
-        ebar[2][2];
+        ebar[2][2], drain;
     uint32_t tmem_base;
-    int abort;
+    int abort, issued_w, issued_z;  // issued: copies the producer asked for
 };
 
 // insertion into the sorted list as a branch-free compare-exchange down the list
@@ -1276,6 +1284,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) lmhead_wide_kernel(const LmHe
             mbar_init(&st.ebar[i][0], 4);
             mbar_init(&st.ebar[i][1], 4);
         }
+        mbar_init(&st.drain, 1);
         st.abort = 0;
         mbar_fence_init();
     }
@@ -1312,7 +1321,8 @@ __global__ void __launch_bounds__(kWideThreads, 1) lmhead_wide_kernel(const LmHe
             // c + SZ and its weight slot iteration c + SW
             int cw = 0, cz = 0;  // c % SW, c % SZ
             uint32_t pd = 0;     // phase bit of done[cw]
-            for (int c = 0; c + SZ < total; ++c) {
+            int c = 0;
+            for (; c + SZ < total; ++c) {
                 if (!mbar_wait_abortable(&st.done[cw], pd, a.status, &st.abort)) break;
                 mbar_arrive_expect_tx(&st.zfull[cz], zbytes);
                 bulk_g2s(zring + (size_t)cz * zbytes, Zsrc + (size_t)kz * zbytes, zbytes, &st.zfull[cz]);
@@ -1324,6 +1334,8 @@ __global__ void __launch_bounds__(kWideThreads, 1) lmhead_wide_kernel(const LmHe
                 if (++cz == SZ) cz = 0;
                 if (++cw == SW) { cw = 0; pd ^= 1u; }
             }
+            st.issued_w = min(c + SW, total);
+            st.issued_z = min(c + SZ, total);
         }
     } else if (warp == 9) {  // ---- MMA issuer
         if (lane == 0) {
@@ -1354,6 +1366,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) lmhead_wide_kernel(const LmHe
                 if (!ok) break;
                 tc_commit(&st.tfull[buf]);
             }
+            if (*(volatile int*)&st.abort) drain_mmas(&st.drain, a.status);
         }
     } else if ((warp >> 2) < ngroups) {  // ---- epilogue warps of row group g = warp / 4
         const int g = warp >> 2, qd = warp & 3;  // row group; TMEM lane quadrant 32 qd .. 32 qd + 31
@@ -1435,6 +1448,10 @@ __global__ void __launch_bounds__(kWideThreads, 1) lmhead_wide_kernel(const LmHe
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (t == 0 && *(volatile int*)&st.abort) {
+        drain_copies(st.wfull, SW, st.issued_w, a.status);
+        drain_copies(st.zfull, SZ, st.issued_z, a.status);
+    }
     if (warp == 0) tc_dealloc(tmem, tmem_cols);
 }
 

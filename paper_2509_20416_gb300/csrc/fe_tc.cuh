@@ -134,4 +134,17 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, float* v) {
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// ---- leaving after a wait of the CTA gave up ------------------------------------------------
+// Never with copies or MMAs in flight: shared memory and tensor memory go to other CTAs.
+// `issued` copies into a ring of S slots, the i-th completing phase i / S of full[i % S]:
+__device__ __forceinline__ void drain_copies(uint64_t* full, int S, int issued, int* status) {
+    for (int i = max(0, issued - S); i < issued; ++i) mbar_wait(&full[i % S], (uint32_t)(i / S) & 1u, status, 100000000LL);
+}
+
+// the calling thread's MMAs; bar: initialised for one arrival, used for nothing else
+__device__ __forceinline__ void drain_mmas(uint64_t* bar, int* status) {
+    tc_commit(bar);
+    mbar_wait(bar, 0u, status, 100000000LL);
+}
+
 }  // namespace fe
