@@ -243,9 +243,10 @@ __global__ void __launch_bounds__(kVsThreads) verify_sampled_kernel(const Verify
 //     depend on their order, so the totals of CTAs, segments and entries agree to the last
 //     bit and the draw never falls between two of them.
 // 4 sequences, 128256 entries, 6 levels x 8 candidates: 324 us on one CTA each; here 28 us with
-// the totals added in double by one warp between CTA barriers, 25.3 with every total a float
-// pair (whose CDF could pick an entry next to its own, even one of probability 0, when the
-// deviate lay within 2^-48 of a CDF edge), 25.9 in fixed point.
+// the totals added in double by one warp between CTA barriers, 25 with every total a float pair
+// (whose CDF could pick an entry next to its own, even one of probability 0, when the deviate
+// lay within 2^-48 of a CDF edge), as much in fixed point (four seeds, one box: 26.6, 26.6, 31.4,
+// 29.4 us in pairs, 25.9, 25.9, 31.1, 28.7 in fixed point).
 struct FF {  // an unevaluated sum of two floats
     float h = 0.f, l = 0.f;
 };
@@ -282,15 +283,19 @@ __device__ __forceinline__ fx64 fx(float w) {
 
 __device__ __forceinline__ fx64 fx_add(fx64 a, fx64 b) { return a + b < a ? ~0ull : a + b; }
 
-// 1 / (a 2^-62), a > 0, rounded once from a remainder known to ~2^-49: a is split into three
-// floats, and the remainder of the first one's reciprocal is exact
+// 1 / (a 2^-62), 0 < a <= kFxOne, rounded once from a remainder known to ~2^-48: a = M 2^(64 - s) with
+// M in [1/2, 1) split into 24 + 24 + 16 bits, and the remainder of the first part's reciprocal
+// is exact. (Conversions of 32-bit words: those of 64-bit ones run at a fraction of the rate, and
+// every warp forms this for every rejection.)
 __device__ __forceinline__ float fx_rcp(fx64 a) {
-    constexpr float kUnit = 1.f / (float)kFxOne;
-    const float h = __ull2float_rn(a);
-    const long long d = (long long)(a - __float2ull_rn(h));  // (|d| < 2^39)
-    const float l = __ll2float_rn(d), l2 = __ll2float_rn(d - __float2ll_rn(l));
-    const float r = __frcp_rn(h * kUnit);
-    return fmaf(r, fmaf(-r, l2 * kUnit, fmaf(-r, l * kUnit, fmaf(-r, h * kUnit, 1.f))), r);
+    const int s = __clzll((long long)a);
+    const fx64 m = a << s;
+    const float h = __uint2float_rn((uint32_t)(m >> 40)) * 0x1p-24f;
+    const float l = __uint2float_rn((uint32_t)(m >> 16) & 0xffffffu) * 0x1p-48f;
+    const float l2 = __uint2float_rn((uint32_t)m & 0xffffu) * 0x1p-64f;
+    const float r = __frcp_rn(h);
+    const float q = fmaf(r, fmaf(-r, l2, fmaf(-r, l, fmaf(-r, h, 1.f))), r);
+    return q * __uint_as_float((uint32_t)(s - 2 + 127) << 23);  // (a 2^-62 = M 2^(2 - s))
 }
 
 // Transposing warp reduction: afterwards lane l holds, in v[0], the warp-wide sum of value
