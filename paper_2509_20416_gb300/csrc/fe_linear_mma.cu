@@ -522,7 +522,14 @@ __global__ void __launch_bounds__(lin_threads(NS), 1) linear_mma_kernel(const Li
         }
     } else if (TM && warp >= 5) {  // ---- MMA issuers: warps 5 and 6 take alternate units
         // (one thread needs ~850 cycles for a unit's waits, four MMAs and commits, more than
-        // the ~680 a unit takes to arrive; the chains are independent, so two threads overlap)
+        // the ~680 a unit takes to arrive; the chains are independent, so two threads overlap.
+        // With an odd number of slots or accumulators an issuer meets each of them at every other
+        // use only, the other issuer's uses between; no wait can take the phase before last for
+        // its own all the same. tempty[buf] of unit `it` follows the drain of unit it - NA, and
+        // units are drained in order: so every unit up to it - NA has arrived, it - S among them
+        // (NA <= S: launch_bp), and full[slot] is in the phase of unit `it`. And before, this
+        // issuer waited for the drain of it - 2 - NA, so that of it - 2 NA (NA >= 2) is done and
+        // tempty[buf] is in the phase that the drain of it - NA completes.)
         if (lane == 0) {
             const uint32_t idesc = idesc_bf16_f32(128, N);
             const int total = (int)(u1 - u0);
@@ -762,7 +769,7 @@ cudaError_t launch_bp(const LinearArgs& a, uint16_t* xb, float* part, int* count
     const size_t budget = (size_t)dev.max_smem_optin - sizeof(LinMmaState) - 1024 - 1024;
     int S = (int)(budget / stage_bytes);
     S = S > kLinMaxStages ? kLinMaxStages : S;
-    if (S < 2) return cudaErrorInvalidValue;
+    if (S < 2 || (NS == 3 && S < acc_buffers(N, NS, MT))) return cudaErrorInvalidValue;
     const size_t smem = 1024 + (size_t)S * stage_bytes;
     uint32_t cols = 32;
     while (cols < (uint32_t)(acc_buffers(N, NS, MT) * MT * N)) cols <<= 1;
