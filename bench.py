@@ -69,15 +69,15 @@ TRAFFIC = {
     # ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum -k regex:linear_kernel
     #     -s 18 -c 6 on `bench.py --workload l33_70b --set n_layers=1 --also ...` (one draft's six linear
     # launches: W_fuse, W_in, W_qkv, W_o, W_gate/up, W_down; the eight-layer draft repeats the last four)
-    "l33_70b": {"bytes_per_draft": (402810112 + 2523392) + (268570624 + 48128)
-                + 8 * ((167917056 + 95744) + (134362624 + 686592) + (939683584 + 122880) + (470004736 + 62208)),
-                "sources": ("fe_stream.cuh", "fe_linear.cu", "fe_common.cuh"), "src": "bdcfc4bf8ebead3c"},
+    "l33_70b": {"bytes_per_draft": (402789632 + 2808576) + (268570624 + 119296)
+                + 8 * ((167903744 + 427776) + (134361344 + 46080) + (939686144 + 128768) + (470043136 + 135936)),
+                "sources": ("fe_stream.cuh", "fe_linear.cu", "fe_common.cuh"), "src": "c4ea127a6d12f2a6"},
     # the same metrics with -k regex:linear_mma_kernel -s 18 -c 6 on `bench.py --workload b32_l31 --set
     # n_layers=1 --also ...` (the tensor-core products of the six phases; the six-layer draft repeats
     # the last four)
-    "b32_l31": {"bytes_per_draft": (102312704 + 2831872) + (68231936 + 17664)
-                + 6 * ((50930432 + 0) + (34153472 + 0) + (235487488 + 2004736) + (119888896 + 385536)),
-                "sources": ("fe_linear_mma.cu", "fe_tc.cuh", "fe_common.cuh"), "src": "7e25be4fcd2f8fe4"},
+    "b32_l31": {"bytes_per_draft": (102321152 + 2927872) + (68233984 + 9216)
+                + 6 * ((50932480 + 0) + (34154752 + 0) + (235489792 + 2273280) + (119892480 + 75008)),
+                "sources": ("fe_linear_mma.cu", "fe_tc.cuh", "fe_common.cuh"), "src": "a5313e108e114ed2"},
 }
 
 

@@ -6,7 +6,7 @@
 // streaming kernel's exact order of additions. The streaming kernel itself holds a whole
 // activation row per batch row in shared memory (8 rows of 16 KB at most), streams the weights
 // once per such tile and reads 2 KB of activations per 512 bytes of weights and lane group: 56
-// rows of an 8B-shaped two-layer draft took 4470 us of linear phases.
+// rows of an 8B-shaped two-layer draft took 4470 us of linear phases, 4750 in all.
 //
 // The order (linear_kernel): the columns of a row are cut into slices of 1024; slice ks of group
 // g goes to warp (phase + ks) % 8 of its CTA; lane l of a warp runs one FMA chain over the
@@ -21,14 +21,14 @@
 //   - Warp w of each of two warp groups (16 rows of weights each) takes chunk w of every block,
 //     i.e. the chains of lanes w, w + 8, w + 16, w + 24; its lanes are 4 weight rows x 8 batch
 //     rows, each lane 4 x NB outputs in registers. A block's loads are broadcasts (one
-//     shared-memory wavefront each): 18 per 224 multiply-adds at 56 rows.
+//     shared-memory wavefront each): 22 per 224 multiply-adds at 56 rows.
 //   - Blocks come in the order of the chains: lane quarter by quarter (0, 2, 1, 3), so that the
 //     butterfly's first two steps are register additions; its last three go through a small
 //     exchange buffer once per class, and the classes' sums are added in warp order at the end.
-// Bound by issue: at 56 rows a warp's 224 multiply-adds of a block (128 instructions, 96 of them
-// two-wide) come with ~64 to widen weights, 26 loads and ~90 of ring, class and loop overhead, at
-// 62 % of the issue rate (57 % of the FMA pipe). Gate/up of the 8B shape at 56 rows (235 MB):
-// streaming kernel 663 us, here 369; one-wide FMAs 450. The draft above: 4750 -> 2247 us.
+// Bound by issue: at 56 rows a warp executes 312 instructions a block, 128 for the 224 multiply-adds
+// (96 two-wide, 32 one-wide), 64 to widen weights, 22 for the loads above and ~98 of ring, class and
+// loop overhead, and issues in 64 % of the cycles. Gate/up of the 8B shape at 56 rows (235 MB):
+// streaming kernel 663 us, here 369; one-wide FMAs 450. The whole draft above: 4750 -> 2247 us.
 #include <algorithm>
 
 #include "fe_kernels.h"
