@@ -126,10 +126,12 @@ typedef struct {
  *             (Steele, Lea and Flood 2014). The drawn set is reported ordered by logit like
  *             the greedy candidates (descending, ties to the smaller id), so the tree rule is
  *             unchanged: the most probable drawn token is the backbone.
- * A sequence's results depend on the others of its call in the last bits of float32: which kernel
- * takes a product, and with it the order of its additions, goes by B (and, up to 8 and from 33
- * sequences, by N B), so the same sequence drafted in calls of different B agrees to a few
- * 1e-7 of its hidden states, not bit for bit. The same call with the same inputs repeats exactly.
+ * A sequence's results depend on the size of its call. Handles of up to 8 and of 33 to 64 sequences
+ * choose the kernel of a product, and with it the order of its additions, by B and N B, so the
+ * same sequence drafted in calls of different B agrees to a few 1e-7 of its hidden states, not
+ * bit for bit; and above 16 hidden rows (N B) the LM head rounds its bf16 handles' normalised
+ * hidden states to bf16, which moves logits by a few 1e-3. The same call with the same inputs
+ * repeats exactly.
  * Outputs (device, float32 unless stated):
  *  topk_id [B, N, top_k] int32, topk_logit [B, N, top_k], topk_prob [B, N, top_k], lse [B, N]
  *  topk_rank [B, N, top_k] int32 or NULL: each candidate's position in draw order (0 =
